@@ -178,6 +178,8 @@ int make_view(const pcas_vol* vol, const pcas_cb* cb, double step, View* V) {
     V->nu = cb->nu;
     V->nv = cb->nv;
     V->step = (float)step;
+    // symmetric to within the rounding of the float geometry
+    V->zsym = fabs(cb->off_v) <= 1e-9 * cb->dv && fabs(vol->oz + 0.5 * (vol->nz - 1) * vol->sz) <= 1e-9 * vol->sz;
     V->swap = 0;                            // launch shapes: set_layouts
     V->lw1 = V->lw4 = 3;
     V->chunk1 = 0;
@@ -1396,10 +1398,10 @@ __global__ void k_ctrl_start(SolveState* st, cudaGraphConditionalHandle h_outer)
     cudaGraphSetConditional(h_outer, (st->max_iter > 0 && st->phase < PH_STOP) ? 1u : 0u);
 }
 
-// End of an iteration (residual, three gradient kernels -- the last of which
+// End of an iteration (residual, four gradient kernels -- one of the last two
 // opened the batch loop -- the batches, and this kernel).
 __global__ void k_ctrl_iter_end(SolveState* st, cudaGraphConditionalHandle h_outer) {
-    st->launches += 5;
+    st->launches += 6;
     int ph = st->phase;
     if (ph == PH_RUNNING) {          // batch cap reached without a decision: end the solve
         ph = PH_STOP;
