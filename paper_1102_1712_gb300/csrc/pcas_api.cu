@@ -3,6 +3,7 @@
 // solve loop of the Appendix, and the small kernels (state set-up, tumour
 // localisation of Sec. II.A).
 #include <math.h>
+#include <stddef.h>
 #include <stdarg.h>
 #include <stdio.h>
 #include <string.h>
@@ -475,6 +476,7 @@ __global__ void k_init_state(SolveState* st, int K, double w0, double w1, double
     st->cur = 0; st->phase = PH_RUNNING; st->evals = 0; st->trials = 0;
     st->nvalid = 0; st->iters = 0; st->batches = 0; st->max_iter = max_iter; st->launches = 0;
     st->wide = 1;
+    st->dense = -1;
     st->jac_ready = 0;
     for (int i = 0; i < 4; i++) st->counter[i] = 0u;
     for (int i = 0; i < 2; i++)
@@ -543,7 +545,7 @@ int eval_gradient_pipeline(const void* f0, const void* mean, const void* U, int 
     PCAS_LAUNCH(PCAS_K_RESID, s, launch_resid(W.pbuf, y, V, W.view, 1, W.rayt, W.st, W.part_res, s));
     PCAS_LAUNCH(PCAS_K_ADJ_GRAD, s,
                 launch_adjoint_grad(W.rayt, g, W.view, W.f0h, occ_of(W, T).f0m, mean, U, dt, K, step_setup, W.st,
-                                    W.part_adj, W.adj, T.vt, gather_blocks(T), 0ull, 0, nullptr, s));
+                                    W.part_adj, W.adj, T.vt, gather_blocks(T), 0ull, 0, nullptr, GradRun{false, -1}, s));
     return PCAS_OK;
 }
 
@@ -566,12 +568,15 @@ int solve_host(const void* f0, const void* mean, const void* U, int dtype, int K
     PCAS_LAUNCH(PCAS_K_DRR_SOLVER, s,
                 launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, 0, W.st, W.part_drr, T, 0ull, 0,
                                   occ_of(W, T), s));
-    int iters = 0, phase = PH_RUNNING;
+    int iters = 0, flags[2] = {PH_RUNNING, -1};      // SolveState::phase, dense
+    int& phase = flags[0];
+    static_assert(offsetof(SolveState, dense) == offsetof(SolveState, phase) + sizeof(int), "read back together");
     for (int it = 0; it < prm->max_iter; it++) {
         PCAS_LAUNCH(PCAS_K_RESID, s, launch_resid(W.pbuf, y, V, W.view, it == 0, W.rayt, W.st, W.part_res, s));
         PCAS_LAUNCH(PCAS_K_ADJ_GRAD, s,
                     launch_adjoint_grad(W.rayt, g, W.view, W.f0h, occ_of(W, T).f0m, mean, U, dtype, K, 1, W.st,
-                                        W.part_adj, W.adj, T.vt, adj_blocks, 0ull, 0, nullptr, s));
+                                        W.part_adj, W.adj, T.vt, adj_blocks, 0ull, 0, nullptr, GradRun{it > 0, flags[1]},
+                                        s));
         // Armijo backtracking over the schedule mu0, beta mu0, ...: the next
         // step sizes that the rule may still try (up to five, two after an
         // iteration that took its first one) are rendered and tested in one
@@ -584,7 +589,7 @@ int solve_host(const void* f0, const void* mean, const void* U, int dtype, int K
             PCAS_LAUNCH(PCAS_K_DRR_BATCH, s,
                         launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, TRIAL_BATCH, W.st, W.part_drr,
                                           T, 0ull, 0, occ_of(W, T), s));
-            PCAS_CUDA(cudaMemcpyAsync(&phase, &W.st->phase, sizeof(int), cudaMemcpyDeviceToHost, s));
+            PCAS_CUDA(cudaMemcpyAsync(flags, &W.st->phase, sizeof(flags), cudaMemcpyDeviceToHost, s));
             PCAS_CUDA(cudaStreamSynchronize(s));
             if (phase != PH_RUNNING) break;
         }
@@ -830,7 +835,7 @@ int cost_grad_f0(const float* f0, const float* mean, const float* U, int K, cons
     if (dJdw)
         PCAS_LAUNCH(PCAS_K_ADJ_GRAD, s,
                     launch_adjoint_grad(W.rayt, g, W.view, W.f0h, occ_of(W, T).f0m, mean, U, DT_F32, K, 0, W.st,
-                                        W.part_adj, W.adj, T.vt, gather_blocks(T), 0ull, 0, nullptr, s));
+                                        W.part_adj, W.adj, T.vt, gather_blocks(T), 0ull, 0, nullptr, GradRun{false, -1}, s));
     if (dJdf0)
         PCAS_LAUNCH(PCAS_K_GRAD_F0, s, launch_grad_f0(W.rayt, g, W.view, mean, U, K, W.st, z, zmax, acc, dJdf0, s));
     SolveState h;
@@ -1386,6 +1391,7 @@ __global__ void k_init_dev(SolveState* st, const InitBlock* __restrict__ ib, con
     st->cur = 0; st->phase = PH_RUNNING; st->evals = 0; st->trials = 0;
     st->nvalid = 0; st->iters = 0; st->batches = 0; st->launches = 1;
     st->wide = 1;
+    st->dense = -1;
     st->jac_ready = 0;
     for (int i = 0; i < 4; i++) st->counter[i] = 0u;
     for (int i = 0; i < 2; i++)
@@ -1599,7 +1605,7 @@ int capture_solve(pcas_solver s, cudaGraph_t graph, cudaStream_t cs, const float
     PCAS_G(launch_resid(W.pbuf, s->y, V, W.view, -1, W.rayt, W.st, W.part_res, cs2));
     PCAS_G(cudaEventRecord(ev_join, cs2));
     PCAS_G(launch_adjoint_grad(W.rayt, g, W.view, W.f0h, oc.f0m, s->mean, s->U, s->dtype, s->K, 1, W.st, W.part_adj,
-                               W.adj, s->tune.vt, gather_blocks(s->tune), s->h_inner, 1, ev_join, cs));
+                               W.adj, s->tune.vt, gather_blocks(s->tune), s->h_inner, 1, ev_join, GradRun{true, -1}, cs));
     cudaGraph_t inner_body;
     PCAS_TRY(add_while(cs, s->h_inner, &inner_body));
     k_ctrl_iter_end<<<1, 1, 0, cs>>>(W.st, s->h_outer);
