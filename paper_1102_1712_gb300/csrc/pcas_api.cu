@@ -540,8 +540,8 @@ int eval_gradient_pipeline(const void* f0, const void* mean, const void* U, int 
     PCAS_TRY(stage_f0h(f0, dt, g, W, T, s));
     PCAS_LAUNCH(PCAS_K_WARP_PCA, s, first_warp(W, T, g, mean, U, dt, K, s));
     PCAS_LAUNCH(PCAS_K_DRR_SOLVER, s,
-                launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, 0, W.st, W.part_drr, T, 0ull, 0,
-                                  occ_of(W, T), s));
+                launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, 0, W.st, W.part_drr, W.part_adj,
+                                  T, 0ull, 0, occ_of(W, T), s));
     PCAS_LAUNCH(PCAS_K_RESID, s, launch_resid(W.pbuf, y, V, W.view, 1, W.rayt, W.st, W.part_res, s));
     PCAS_LAUNCH(PCAS_K_ADJ_GRAD, s,
                 launch_adjoint_grad(W.rayt, g, W.view, W.f0h, occ_of(W, T).f0m, mean, U, dt, K, step_setup, W.st,
@@ -566,8 +566,8 @@ int solve_host(const void* f0, const void* mean, const void* U, int dtype, int K
     PCAS_TRY(stage_f0h(f0, dtype, g, W, T, s));
     PCAS_LAUNCH(PCAS_K_WARP_PCA, s, first_warp(W, T, g, mean, U, dtype, K, s));
     PCAS_LAUNCH(PCAS_K_DRR_SOLVER, s,
-                launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, 0, W.st, W.part_drr, T, 0ull, 0,
-                                  occ_of(W, T), s));
+                launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, 0, W.st, W.part_drr, W.part_adj,
+                                  T, 0ull, 0, occ_of(W, T), s));
     int iters = 0, flags[2] = {PH_RUNNING, -1};      // SolveState::phase, dense
     int& phase = flags[0];
     static_assert(offsetof(SolveState, dense) == offsetof(SolveState, phase) + sizeof(int), "read back together");
@@ -587,8 +587,8 @@ int solve_host(const void* f0, const void* mean, const void* U, int dtype, int K
             PCAS_LAUNCH(PCAS_K_WARP_BATCH, s, launch_warp_batch(W.f0h, mean, U, dtype, K, W.st, g, W.view,
                                                                 W.fpad4, W.fpad, occ_of(W, T), s));
             PCAS_LAUNCH(PCAS_K_DRR_BATCH, s,
-                        launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, TRIAL_BATCH, W.st, W.part_drr,
-                                          T, 0ull, 0, occ_of(W, T), s));
+                        launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, TRIAL_BATCH, W.st,
+                                          W.part_drr, W.part_adj, T, 0ull, 0, occ_of(W, T), s));
             PCAS_CUDA(cudaMemcpyAsync(flags, &W.st->phase, sizeof(flags), cudaMemcpyDeviceToHost, s));
             PCAS_CUDA(cudaStreamSynchronize(s));
             if (phase != PH_RUNNING) break;
@@ -829,8 +829,8 @@ int cost_grad_f0(const float* f0, const float* mean, const float* U, int K, cons
         PCAS_LAUNCH(PCAS_K_WARP_PCA, s, launch_warp_pca(W.f0h, mean, U, DT_F32, K, wsrc, g, W.view, W.fpad,
                                                         pair_of(W, T), W.st->box[0], occ_of(W, T), s));
     PCAS_LAUNCH(PCAS_K_DRR_SOLVER, s,
-                launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, 0, W.st, W.part_drr, T, 0ull, 0,
-                                  occ_of(W, T), s));
+                launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, 0, W.st, W.part_drr, W.part_adj,
+                                  T, 0ull, 0, occ_of(W, T), s));
     PCAS_LAUNCH(PCAS_K_RESID, s, launch_resid(W.pbuf, y, V, W.view, 1, W.rayt, W.st, W.part_res, s));
     if (dJdw)
         PCAS_LAUNCH(PCAS_K_ADJ_GRAD, s,
@@ -1586,8 +1586,8 @@ int capture_solve(pcas_solver s, cudaGraph_t graph, cudaStream_t cs, const float
     // projection of a run (k_init_dev sets keep_f0h then)
     PCAS_G(launch_fill_f0h(s->f0, s->dtype, g, W.f0h, s->tune.skip ? W.f0m : nullptr, &W.st->keep_f0h, cs));
     PCAS_G(first_warp(W, s->tune, g, s->mean, s->U, s->dtype, s->K, cs));
-    PCAS_G(launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, s->y, W.pbuf, 0, W.st, W.part_drr, s->tune, 0ull, 0,
-                             oc, cs));
+    PCAS_G(launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, s->y, W.pbuf, 0, W.st, W.part_drr, W.part_adj,
+                             s->tune, 0ull, 0, oc, cs));
     k_ctrl_start<<<1, 1, 0, cs>>>(W.st, s->h_outer);
     PCAS_G(cudaGetLastError());
     cudaGraph_t outer_body;
@@ -1616,7 +1616,7 @@ int capture_solve(pcas_solver s, cudaGraph_t graph, cudaStream_t cs, const float
     PCAS_G(cudaStreamBeginCaptureToGraph(cs, inner_body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
     PCAS_G(launch_warp_batch(W.f0h, s->mean, s->U, s->dtype, s->K, W.st, g, W.view, W.fpad4, W.fpad, oc, cs));
     PCAS_G(launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, s->y, W.pbuf, TRIAL_BATCH, W.st, W.part_drr,
-                             s->tune, s->h_inner, 1, oc, cs));
+                             W.part_adj, s->tune, s->h_inner, 1, oc, cs));
     PCAS_G(cudaStreamEndCapture(cs, &done));
     return PCAS_OK;
 }
