@@ -239,7 +239,7 @@ struct Ws {
     View* view;
     float* f0h;
     unsigned char* f0m;       // bricks of the reference CT, right after f0h
-    size_t f0h_bytes;         // f0h and f0m
+    size_t f0h_bytes, f0m_bytes;      // f0h and f0m; f0m alone
     unsigned int* occ;        // occupancy bricks of the solver volumes
     float *fpad, *pbuf;
     float2* fpair;
@@ -261,6 +261,7 @@ int bind_ws(void* ws, size_t ws_bytes, const pcas_vol* vol, const pcas_cb* cb, i
     W->f0h = reinterpret_cast<float*>(b + L.f0h);
     W->f0m = reinterpret_cast<unsigned char*>(b + L.f0m);
     W->f0h_bytes = L.fpad - L.f0h;
+    W->f0m_bytes = L.fpad - L.f0m;
     W->fpad = reinterpret_cast<float*>(b + L.fpad);
     W->fpair = reinterpret_cast<float2*>(b + L.fpair);
     W->fpad4 = reinterpret_cast<float4*>(b + L.fpad4);
@@ -454,53 +455,6 @@ __global__ void k_localize(const T* __restrict__ mean, const T* __restrict__ U, 
     localize_warp(mean, U, K, g, w, ox, oy, oz, isx, isy, isz, cx, cy, cz, max_iter, tol, out);
 }
 
-// Reset the solver state for a new evaluation/solve.
-__global__ void k_init_state(SolveState* st, int K, double w0, double w1, double w2, double w3,
-                             double w4, double w5, double w6, double w7, double mu0, double alpha,
-                             double beta, double mu_min, int max_trials, int max_iter) {
-    if (threadIdx.x != 0) return;
-    const double w[PCAS_KMAX] = {w0, w1, w2, w3, w4, w5, w6, w7};
-    for (int k = 0; k < PCAS_KMAX; k++) {
-        st->w[k] = k < K ? w[k] : 0.0;
-        st->d[k] = 0.0;
-        st->G[k] = 0.0;
-        for (int j = 0; j < TRIAL_BATCH; j++) st->wt[j][k] = st->w[k];
-    }
-    for (int j = 0; j < TRIAL_BATCH; j++) st->mu_batch[j] = 0.0;
-    st->gnorm = st->a = st->b = st->J = st->J0 = st->Jt = 0.0;
-    st->mu = mu0;
-    for (int i = 0; i < NBUF; i++)
-        for (int j = 0; j < NMOM; j++) st->mom[i][j] = 0.0;
-    st->mu0 = mu0; st->alpha = alpha; st->beta = beta; st->mu_min = mu_min;
-    st->K = K; st->max_trials = max_trials;
-    st->cur = 0; st->phase = PH_RUNNING; st->evals = 0; st->trials = 0;
-    st->nvalid = 0; st->iters = 0; st->batches = 0; st->max_iter = max_iter; st->launches = 0;
-    st->wide = 1;
-    st->dense = -1;
-    st->jac_ready = 0;
-    for (int i = 0; i < 4; i++) st->counter[i] = 0u;
-    for (int i = 0; i < 2; i++)
-        for (int j = 0; j < 6; j++) st->box[i][j] = BOX_EMPTY;
-}
-
-int upload_view(View* dst, const View& V, cudaStream_t s) {
-    PCAS_CUDA(cudaMemcpyAsync(dst, &V, sizeof(View), cudaMemcpyHostToDevice, s));
-    return PCAS_OK;
-}
-
-int launch_init(SolveState* st, int K, const double* w, const pcas_params* prm, cudaStream_t s) {
-    double v[PCAS_KMAX] = {0};
-    for (int k = 0; k < K; k++) v[k] = w[k];
-    pcas_params d = {0.2, 0.1, 0.5, 0.01, 10, 30, 1.0};
-    if (!prm) prm = &d;
-    PCAS_LAUNCH(PCAS_K_INIT, s,
-                (k_init_state<<<1, 32, 0, s>>>(st, K, v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7],
-                                               prm->mu0, prm->alpha, prm->beta, prm->mu_min,
-                                               prm->max_trials, prm->max_iter),
-                 cudaGetLastError()));
-    return PCAS_OK;
-}
-
 int check_dtype(int dt) {
     if (dt != PCAS_F32 && dt != PCAS_BF16 && dt != PCAS_F16)
         return fail(PCAS_ERR_INVALID_ARG, "storage dtype must be PCAS_F32, PCAS_BF16 or PCAS_F16, got %d", dt);
@@ -524,10 +478,108 @@ int check_finite(const double* v, int n, const char* name) {
         if (rc_ != PCAS_OK) return rc_; \
     } while (0)
 
-// The halo copy of the reference CT for this call and its bricks (zeroed,
-// then filled).
+// The start of an evaluation or solve, in one launch: the solver state, the
+// view, the reference CT's bricks and the halos of the solver volumes (whose
+// interior the warps write whole).  Zeroing the volumes whole took 20 us at
+// 256x256x100 and 110 us at 512x512x160; the halos, the state and the view
+// (separate launches and copies before) take 5 and 12.
+struct HaloRows {             // a volume of rows pitch floats long: interior [lo, hi) in rows
+    float* p;                 // 2 <= j < ny + 2, 2 <= k < nz + 2 of pny x pnz
+    int pitch, lo, hi;
+};
+struct Prepare {
+    double w[PCAS_KMAX], mu0, alpha, beta, mu_min;
+    int K, max_trials, max_iter;
+    View view;
+    View* view_out;
+    HaloRows vol[3];
+    int nvol, ny, nz;
+    unsigned int* bricks;     // words to zero (a multiple of 4 bytes)
+    int nbricks;
+};
+__device__ void init_state(SolveState* st, const Prepare& p) {
+    for (int k = 0; k < PCAS_KMAX; k++) {
+        st->w[k] = k < p.K ? p.w[k] : 0.0;
+        st->d[k] = 0.0;
+        st->G[k] = 0.0;
+        for (int j = 0; j < TRIAL_BATCH; j++) st->wt[j][k] = st->w[k];
+    }
+    for (int j = 0; j < TRIAL_BATCH; j++) st->mu_batch[j] = 0.0;
+    st->gnorm = st->a = st->b = st->J = st->J0 = st->Jt = 0.0;
+    st->mu = p.mu0;
+    for (int i = 0; i < NBUF; i++)
+        for (int j = 0; j < NMOM; j++) st->mom[i][j] = 0.0;
+    st->mu0 = p.mu0; st->alpha = p.alpha; st->beta = p.beta; st->mu_min = p.mu_min;
+    st->K = p.K; st->max_trials = p.max_trials;
+    st->cur = 0; st->phase = PH_RUNNING; st->evals = 0; st->trials = 0;
+    st->nvalid = 0; st->iters = 0; st->batches = 0; st->max_iter = p.max_iter; st->launches = 0;
+    st->wide = 1;
+    st->dense = -1;
+    st->jac_ready = 0;
+    for (int i = 0; i < 4; i++) st->counter[i] = 0u;
+    for (int i = 0; i < 2; i++)
+        for (int j = 0; j < 6; j++) st->box[i][j] = BOX_EMPTY;
+}
+__global__ void __launch_bounds__(256)
+k_prepare(SolveState* st, const __grid_constant__ Prepare p) {
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) init_state(st, p);
+        if (threadIdx.x == 32) *p.view_out = p.view;
+    }
+    const int threads = gridDim.x * blockDim.x, me = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int t = me; t < p.nbricks; t += threads) p.bricks[t] = 0u;
+    const int lane = threadIdx.x & 31, pny = p.ny + 4, rows = pny * (p.nz + 4);
+#pragma unroll
+    for (int v = 0; v < 3; v++) {
+        if (v >= p.nvol) break;
+        const HaloRows h = p.vol[v];
+        for (int r = me >> 5; r < rows; r += threads >> 5) {
+            const int j = r % pny, k = r / pny;
+            float* __restrict__ row = h.p + (long)r * h.pitch;
+            if (j >= 2 && j < p.ny + 2 && k >= 2 && k < p.nz + 2) {
+                if (lane < h.lo) row[lane] = 0.0f;             // lo <= 16
+                for (int x = h.hi + lane; x < h.pitch; x += 32) row[x] = 0.0f;
+            } else {
+                float4* __restrict__ row4 = reinterpret_cast<float4*>(row);     // rows are multiples of 16 bytes
+                for (int x = lane; x < h.pitch / 4; x += 32) row4[x] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
+        }
+    }
+}
+
+// batch: also the volumes of the line search (f and the candidates; the first
+// evaluation alone uses the x pairs).
+int prepare(const Ws& W, const View& V, const Grid& g, int K, const double* w, const pcas_params* prm, bool skip,
+            bool batch, cudaStream_t s) {
+    Prepare p{};
+    for (int k = 0; k < K; k++) p.w[k] = w[k];
+    const pcas_params d = {0.2, 0.1, 0.5, 0.01, 10, 30, 1.0};
+    if (!prm) prm = &d;
+    p.mu0 = prm->mu0; p.alpha = prm->alpha; p.beta = prm->beta; p.mu_min = prm->mu_min;
+    p.K = K; p.max_trials = prm->max_trials; p.max_iter = prm->max_iter;
+    p.view = V;
+    p.view_out = W.view;
+    const Pad pd = solver_pad(g.nx, g.ny, g.nz, V.swap);
+    const int nx = V.swap ? g.ny : g.nx;
+    p.ny = V.swap ? g.nx : g.ny;
+    p.nz = g.nz;
+    p.vol[0] = {reinterpret_cast<float*>(W.fpair), 2 * pd.px, 7, 2 * nx + 7};
+    p.vol[1] = {W.fpad, pd.px, 4, nx + 4};
+    p.vol[2] = {reinterpret_cast<float*>(W.fpad4), 4 * pd.px, 16, 4 * (nx + 4)};
+    p.nvol = batch ? 3 : 1;
+    if (skip) {
+        p.bricks = reinterpret_cast<unsigned int*>(W.f0m);
+        p.nbricks = (int)(W.f0m_bytes / 4);
+    }
+    const long rows = (long)pd.pny * pd.pnz, want = (rows + 7) / 8;
+    PCAS_LAUNCH(PCAS_K_INIT, s, (k_prepare<<<(unsigned)(want < 1216 ? want : 1216), 256, 0, s>>>(W.st, p),
+                                 cudaGetLastError()));
+    return PCAS_OK;
+}
+
+// The halo copy of the reference CT for this call and its bricks (zeroed by
+// prepare).
 int stage_f0h(const void* f0, int dt, const Grid& g, const Ws& W, const Tune& T, cudaStream_t s) {
-    PCAS_CUDA(cudaMemsetAsync(W.f0h, 0, W.f0h_bytes, s));
     PCAS_LAUNCH(PCAS_K_INIT, s, launch_fill_f0h(f0, dt, g, W.f0h, T.skip ? W.f0m : nullptr, nullptr, s));
     return PCAS_OK;
 }
@@ -560,9 +612,7 @@ int solve_host(const void* f0, const void* mean, const void* U, int dtype, int K
     PCAS_TRY(bind_ws(ws, ws_bytes, vol, cb, K, &W));
     Grid g = make_grid(vol);
     const int adj_blocks = gather_blocks(T);
-    PCAS_CUDA(cudaMemsetAsync(W.fpad, 0, W.fpad_bytes + W.fpad4_bytes, s));   // zero halos
-    PCAS_TRY(launch_init(W.st, K, w_init, prm, s));
-    PCAS_TRY(upload_view(W.view, V, s));
+    PCAS_TRY(prepare(W, V, g, K, w_init, prm, T.skip != 0, true, s));
     PCAS_TRY(stage_f0h(f0, dtype, g, W, T, s));
     PCAS_LAUNCH(PCAS_K_WARP_PCA, s, first_warp(W, T, g, mean, U, dtype, K, s));
     PCAS_LAUNCH(PCAS_K_DRR_SOLVER, s,
@@ -760,9 +810,7 @@ int cost_grad_typed(const void* f0, const void* mean, const void* U, int dtype, 
     PCAS_TRY(bind_ws(ws, ws_bytes, vol, cb, K, &W));
     cudaStream_t s = as_stream(stream);
     Grid g = make_grid(vol);
-    PCAS_CUDA(cudaMemsetAsync(W.fpad, 0, W.fpad_bytes, s));
-    PCAS_TRY(launch_init(W.st, K, w, nullptr, s));
-    PCAS_TRY(upload_view(W.view, V, s));
+    PCAS_TRY(prepare(W, V, g, K, w, nullptr, T.skip != 0, false, s));
     PCAS_TRY(eval_gradient_pipeline(f0, mean, U, dtype, K, y, g, V, W, 0, T, s));
     SolveState h;
     PCAS_CUDA(cudaMemcpyAsync(&h, W.st, sizeof(h), cudaMemcpyDeviceToHost, s));
@@ -816,9 +864,7 @@ int cost_grad_f0(const float* f0, const float* mean, const float* U, int K, cons
     unsigned int* zmax = reinterpret_cast<unsigned int*>(extra + align256(N * sizeof(float)) + align256(N * 8));
     cudaStream_t s = as_stream(stream);
     Grid g = make_grid(vol);
-    PCAS_CUDA(cudaMemsetAsync(W.fpad, 0, W.fpad_bytes, s));
-    PCAS_TRY(launch_init(W.st, K, w, nullptr, s));
-    PCAS_TRY(upload_view(W.view, V, s));
+    PCAS_TRY(prepare(W, V, g, K, w, nullptr, T.skip != 0, false, s));
     WSrc wsrc{};
     wsrc.dev = W.st->w;
     wsrc.phase = &W.st->phase;

@@ -100,36 +100,49 @@ k_warp_dvf(const T* __restrict__ f0, const float* __restrict__ dvf, Grid g, long
 // i = (blockIdx.x blockDim.x + threadIdx.x) V with V voxels per thread (no
 // index divisions; 32-bit voxel offsets, volumes have < 2^31 voxels).
 
-// The halo copy of the reference CT (see tri_halo): interior only.  With f0m
-// it marks the bricks whose taps include a non-zero voxel (see Occ): voxel i
-// is a tap of the cells of bricks i >> 3 and (i + 1) >> 3 along each axis;
-// one lane per warp marks the span of the warp's non-zero voxels of a row.
-// Blocks stride over the rows (j, k).  skip (may be null): when it holds a
-// non-zero value the copy is current and the kernel returns at once.
+// The halo copy of the reference CT (see tri_halo), halo included: a warp per
+// row, 128 values in flight.  With f0m (zeroed by the caller) it marks the
+// bricks whose taps include a non-zero voxel (see Occ): voxel i is a tap of the
+// cells of bricks i >> 3 and (i + 1) >> 3 along each axis; one lane marks the
+// span of the non-zero voxels among 32 of a row.  skip (may be null): when it
+// holds a non-zero value the copy is current and the kernel returns at once.
+// Bound by HBM: 256x256x100 48 us (interior alone, a block per row, after a
+// memset of 6 us) -> 14 us, 512x512x160 from bfloat16 199 + 26 -> 80 us.
 template <typename T>
 __global__ void __launch_bounds__(kWarpThreads)
 k_fill_f0h(const T* __restrict__ f0, Grid g, float* __restrict__ f0h, unsigned char* __restrict__ f0m,
            const int* __restrict__ skip) {
     if (skip && *skip) return;
-    const long sy = g.nx + 2 * F0_HALO, sz = sy * (g.ny + 2 * F0_HALO);
+    const int px = g.nx + 2 * F0_HALO, py = g.ny + 2 * F0_HALO, rows = py * (g.nz + 2 * F0_HALO);
     const int nbx = f0b_n(g.nx), nby = f0b_n(g.ny);
-    const int rows = g.ny * g.nz;
-    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-        const int j = r % g.ny, k = r / g.ny;
-        for (int i0 = 0; i0 < g.nx; i0 += blockDim.x) {      // the same trip count for every lane
-            const int i = i0 + threadIdx.x;
-            float v = 0.0f;
-            if (i < g.nx) {
-                v = ldg_f(f0 + ((long)k * g.ny + j) * g.nx + i);
-                f0h[(k + F0_HALO) * sz + (j + F0_HALO) * sy + (i + F0_HALO)] = v;
+    const int lane = threadIdx.x & 31, warps = gridDim.x * (kWarpThreads / 32);
+    for (int r = blockIdx.x * (kWarpThreads / 32) + (threadIdx.x >> 5); r < rows; r += warps) {
+        const int j = r % py - F0_HALO, k = r / py - F0_HALO;
+        const bool in = j >= 0 && j < g.ny && k >= 0 && k < g.nz;
+        const T* __restrict__ src = f0 + ((long)k * g.ny + j) * g.nx;
+        float* __restrict__ dst = f0h + (long)r * px;
+        for (int x0 = 0; x0 < px; x0 += 128) {
+            float v[4];
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const int i = x0 + 32 * e + lane - F0_HALO;
+                v[e] = in && i >= 0 && i < g.nx ? ldg_f(src + i) : 0.0f;
             }
-            if (!f0m) continue;
-            const int lo = __reduce_min_sync(0xffffffffu, v != 0.0f ? i : INT_MAX);
-            const int hi = __reduce_max_sync(0xffffffffu, v != 0.0f ? i : INT_MIN);
-            if ((threadIdx.x & 31) != 0 || lo > hi) continue;
-            for (int bz = k >> 3; bz <= (k + 1) >> 3; bz++)
-                for (int by = j >> 3; by <= (j + 1) >> 3; by++)
-                    for (int bx = lo >> 3; bx <= (hi + 1) >> 3; bx++) f0m[(bz * nby + by) * nbx + bx] = 1;
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const int x = x0 + 32 * e + lane;
+                if (x < px) dst[x] = v[e];
+            }
+            if (!f0m || !in) continue;
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const unsigned live = __ballot_sync(0xffffffffu, v[e] != 0.0f);
+                if (lane != 0 || live == 0) continue;
+                const int i = x0 + 32 * e - F0_HALO, lo = i + __ffs((int)live) - 1, hi = i + 31 - __clz((int)live);
+                for (int bz = k >> 3; bz <= (k + 1) >> 3; bz++)
+                    for (int by = j >> 3; by <= (j + 1) >> 3; by++)
+                        for (int bx = lo >> 3; bx <= (hi + 1) >> 3; bx++) f0m[(bz * nby + by) * nbx + bx] = 1;
+            }
         }
     }
 }
@@ -436,8 +449,8 @@ cudaError_t launch_warp_dvf(const void* f0, int dt, const float* dvf, Grid g, fl
 
 cudaError_t launch_fill_f0h(const void* f0, int dt, Grid g, float* f0h, unsigned char* f0m, const int* skip,
                             cudaStream_t s) {
-    const int rows = g.ny * g.nz;
-    const unsigned nb = (unsigned)(rows < 1216 ? rows : 1216);     // 8 blocks per SM of a GB300
+    const int per = kWarpThreads / 32, rows = (g.ny + 2 * F0_HALO) * (g.nz + 2 * F0_HALO), want = (rows + per - 1) / per;
+    const unsigned nb = (unsigned)(want < 1216 ? want : 1216);     // 8 blocks per SM of a GB300
     PCAS_DT_DISPATCH(dt, (k_fill_f0h<T><<<nb, kWarpThreads, 0, s>>>(static_cast<const T*>(f0), g, f0h, f0m, skip),
                           cudaGetLastError()))
 }
