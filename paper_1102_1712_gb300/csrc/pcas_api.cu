@@ -867,7 +867,9 @@ int cost_grad_f0(const float* f0, const float* mean, const float* U, int K, cons
     wsrc.dev = W.st->w;
     wsrc.phase = &W.st->phase;
     PCAS_TRY(stage_f0h(f0, DT_F32, g, W, T, s));
-    if (dJdw)       // the gradient at w follows: its Jacobian pass comes with the warp
+    // the gradient at w follows: its Jacobian pass comes with the warp (and is
+    // left unused where only the rows' alignment asks for this warp)
+    if (dJdw || !warp_pca_fits(mean, U, DT_F32, g))
         PCAS_LAUNCH(PCAS_K_WARP_PCA, s, first_warp(W, T, g, mean, U, DT_F32, K, s));
     else
         PCAS_LAUNCH(PCAS_K_WARP_PCA, s, launch_warp_pca(W.f0h, mean, U, DT_F32, K, wsrc, g, W.view, W.fpad,

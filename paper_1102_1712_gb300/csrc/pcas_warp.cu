@@ -205,8 +205,10 @@ k_fill_f0h(const T* __restrict__ f0, Grid g, float* __restrict__ f0h, unsigned c
 // first value of its own pair and the second of the pair before it; the
 // pairs' halo values stay the zeros the caller wrote); marks the occupancy
 // bricks of its non-zero voxels.
-// VEC: 4 voxels per thread along x (nx % 4 == 0, 16-byte aligned model).
-template <bool VEC, typename T>
+// 4 voxels per thread along x (nx % 4 == 0, 16-byte aligned model; other rows
+// go through launch_warp_jac, whose coalesced single loads take half the time
+// of one voxel a thread here: 149x131x67, K = 2, 46 -> 24 us).
+template <typename T>
 __global__ void __launch_bounds__(kWarpThreads)
 k_warp_pca(const float* __restrict__ f0h, const T* __restrict__ mean,
            const T* __restrict__ U, int K, WSrc ws, Grid g, const View* __restrict__ Vp,
@@ -228,77 +230,49 @@ k_warp_pca(const float* __restrict__ f0h, const T* __restrict__ mean,
     const int j = blockIdx.y, k = blockIdx.z;
     const long N = (long)g.nx * g.ny * g.nz;
     const int row = (k * g.ny + j) * g.nx;
-    if (VEC) {
-        const int i = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
-        if (i < g.nx) {
-            const int n = row + i;
-            float x[3][4];
-            dvf4(mean, U, K, s_w, N, n, x);
-            float o[4];
-            int e0 = 4, e1 = -1;                    // first and last non-zero of the four
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    if (i < g.nx) {
+        const int n = row + i;
+        float x[3][4];
+        dvf4(mean, U, K, s_w, N, n, x);
+        float o[4];
+        int e0 = 4, e1 = -1;                    // first and last non-zero of the four
 #pragma unroll
-            for (int e = 0; e < 4; e++) {
-                o[e] = tri_halo_m(f0h, occ.f0m, g, fmaf(x[0][e], g.inv_sx, (float)(i + e)),
-                                   fmaf(x[1][e], g.inv_sy, (float)j), fmaf(x[2][e], g.inv_sz, (float)k));
-                if (o[e] != 0.0f) {
-                    if (swp) box_add(b, j, i + e, k);
-                    else box_add(b, i + e, j, k);
-                    e0 = min(e0, e);
-                    e1 = e;
-                }
-            }
-            if (oc.m && e1 >= 0) {
-                if (swp) occ_mark(oc.m, oc.gen, oc.nbx, oc.nby, j, j, i + e0, i + e1, k);
-                else occ_mark(oc.m, oc.gen, oc.nbx, oc.nby, i + e0, i + e1, j, j, k);
-            }
-            if (fpair) {                    // voxel d is .x of pair d and .y of pair d - 1
-                float* p = reinterpret_cast<float*>(fpair);
-                if (swp) {
-#pragma unroll
-                    for (int e = 0; e < 4; e++) {
-                        const long d = pad_index(pd, j, i + e, k);
-                        p[2 * d - 1] = o[e];
-                        p[2 * d] = o[e];
-                    }
-                } else {                    // d a multiple of 4: floats 2d - 1 ... 2d + 6
-                    const long d = pad_index(pd, i, j, k);
-                    p[2 * d - 1] = o[0];
-                    *reinterpret_cast<float4*>(p + 2 * d) = make_float4(o[0], o[1], o[1], o[2]);
-                    *reinterpret_cast<float2*>(p + 2 * d + 4) = make_float2(o[2], o[3]);
-                    p[2 * d + 6] = o[3];
-                }
-            } else if (swp) {
-#pragma unroll
-                for (int e = 0; e < 4; e++) fpad[pad_index(pd, j, i + e, k)] = o[e];
-            } else {
-                *reinterpret_cast<float4*>(fpad + pad_index(pd, i, j, k)) = make_float4(o[0], o[1], o[2], o[3]);
+        for (int e = 0; e < 4; e++) {
+            o[e] = tri_halo_m(f0h, occ.f0m, g, fmaf(x[0][e], g.inv_sx, (float)(i + e)),
+                               fmaf(x[1][e], g.inv_sy, (float)j), fmaf(x[2][e], g.inv_sz, (float)k));
+            if (o[e] != 0.0f) {
+                if (swp) box_add(b, j, i + e, k);
+                else box_add(b, i + e, j, k);
+                e0 = min(e0, e);
+                e1 = e;
             }
         }
-    } else {
-        const int i = blockIdx.x * blockDim.x + threadIdx.x;
-        if (i < g.nx) {
-            const int n = row + i;
-            float x[3];
-            for (int c = 0; c < 3; c++) {
-                float v = mean ? ldg_f(mean + c * N + n) : 0.0f;
-                for (int kk = 0; kk < K; kk++) v = fmaf(s_w[kk], ldg_f(U + ((long)kk * 3 + c) * N + n), v);
-                x[c] = v;
+        if (oc.m && e1 >= 0) {
+            if (swp) occ_mark(oc.m, oc.gen, oc.nbx, oc.nby, j, j, i + e0, i + e1, k);
+            else occ_mark(oc.m, oc.gen, oc.nbx, oc.nby, i + e0, i + e1, j, j, k);
+        }
+        if (fpair) {                    // voxel d is .x of pair d and .y of pair d - 1
+            float* p = reinterpret_cast<float*>(fpair);
+            if (swp) {
+#pragma unroll
+                for (int e = 0; e < 4; e++) {
+                    const long d = pad_index(pd, j, i + e, k);
+                    p[2 * d - 1] = o[e];
+                    p[2 * d] = o[e];
+                }
+            } else {                    // d a multiple of 4: floats 2d - 1 ... 2d + 6
+                const long d = pad_index(pd, i, j, k);
+                p[2 * d - 1] = o[0];
+                *reinterpret_cast<float4*>(p + 2 * d) = make_float4(o[0], o[1], o[1], o[2]);
+                *reinterpret_cast<float2*>(p + 2 * d + 4) = make_float2(o[2], o[3]);
+                p[2 * d + 6] = o[3];
             }
-            const float o = tri_halo_m(f0h, occ.f0m, g, fmaf(x[0], g.inv_sx, (float)i),
-                                        fmaf(x[1], g.inv_sy, (float)j), fmaf(x[2], g.inv_sz, (float)k));
-            const int a0 = swp ? j : i, a1 = swp ? i : j;
-            if (o != 0.0f) {
-                box_add(b, a0, a1, k);
-                if (oc.m) occ_mark(oc.m, oc.gen, oc.nbx, oc.nby, a0, a0, a1, a1, k);
-            }
-            const long d = pad_index(pd, a0, a1, k);
-            if (fpair) {
-                float* p = reinterpret_cast<float*>(fpair);
-                p[2 * d - 1] = o;
-                p[2 * d] = o;
-            } else {
-                fpad[d] = o;
-            }
+        } else if (swp) {
+#pragma unroll
+            for (int e = 0; e < 4; e++) fpad[pad_index(pd, j, i + e, k)] = o[e];
+        } else {
+            *reinterpret_cast<float4*>(fpad + pad_index(pd, i, j, k)) = make_float4(o[0], o[1], o[2], o[3]);
         }
     }
     box_reduce(b, box_out);
@@ -454,12 +428,11 @@ template <typename T>
 cudaError_t warp_pca_t(const float* f, const void* mean, const void* U, int K, WSrc w, Grid g,
                        const View* Vd, float* fpad, float2* fpair, int* box, Occ oc, cudaStream_t s) {
     const unsigned a = sizeof(T) * 4;
-    bool vec = (g.nx % 4 == 0) && aligned(mean, a) && aligned(U, a) && aligned(fpad, 16) && aligned(fpair, 16);
-    const T* m = static_cast<const T*>(mean);
-    const T* u = static_cast<const T*>(U);
-    const RowLaunch L = row_launch(g, vec ? 4 : 1);
-    if (vec) k_warp_pca<true, T><<<L.grid, L.threads, 0, s>>>(f, m, u, K, w, g, Vd, fpad, fpair, box, oc);
-    else k_warp_pca<false, T><<<L.grid, L.threads, 0, s>>>(f, m, u, K, w, g, Vd, fpad, fpair, box, oc);
+    if (g.nx % 4 || !aligned(mean, a) || !aligned(U, a) || !aligned(fpad, 16) || !aligned(fpair, 16))
+        return cudaErrorInvalidValue;       // warp_pca_fits
+    const RowLaunch L = row_launch(g, 4);
+    k_warp_pca<T><<<L.grid, L.threads, 0, s>>>(f, static_cast<const T*>(mean), static_cast<const T*>(U), K, w, g, Vd,
+                                               fpad, fpair, box, oc);
     return cudaGetLastError();
 }
 
@@ -505,6 +478,11 @@ cudaError_t launch_fill_f0h(const void* f0, int dt, Grid g, float* f0h, unsigned
     const unsigned nb = (unsigned)(want < 1216 ? want : 1216);     // 8 blocks per SM of a GB300
     PCAS_DT_DISPATCH(dt, (k_fill_f0h<T><<<nb, kWarpThreads, 0, s>>>(static_cast<const T*>(f0), g, f0h, f0m, skip),
                           cudaGetLastError()))
+}
+
+bool warp_pca_fits(const void* mean, const void* U, int dt, const Grid& g) {
+    const unsigned a = dt == DT_F32 ? 16 : 8;
+    return g.nx % 4 == 0 && aligned(mean, a) && aligned(U, a);
 }
 
 cudaError_t launch_warp_pca(const float* f0, const void* mean, const void* U, int dt, int K, WSrc w,
