@@ -109,8 +109,9 @@ int drr_forward(const float* f, const pcas_vol* vol, const pcas_cb* cb, double s
  * source through the pixel centre of the piecewise-constant volume (voxel
  * (i,j,k) = f on the cube of side (sx, sy, sz) centred on it, zero outside).
  * Used to render measured images without the inverse crime of projecting
- * with the solver's own P; not on the solver path.  Voxel traversal and the
- * sum in double precision, p rounded to float.  f, p: device.  Asynchronous.
+ * with the solver's own P; not on the solver path.  Ray geometry in double
+ * precision, voxel traversal in 64-bit fixed point (2^-44 voxel), sums
+ * compensated, p rounded to float once.  f, p: device.  Asynchronous.
  * Errors: PCAS_ERR_INVALID_ARG for a NULL pointer, an invalid volume or
  * view, or a volume not entirely in front of the source. */
 int drr_siddon(const float* f, const pcas_vol* vol, const pcas_cb* cb, float* p, void* stream);
@@ -180,8 +181,8 @@ int cost_grad_static(const float* f0, const float* mean, const float* U, int K, 
  * one projection pass for all of them; two when the previous iteration took
  * its first step size) and tested in schedule order, so the accepted step is
  * the one the one-at-a-time rule would take; stats->evals counts evaluations
- * as that rule would.  Synchronous (one host read of a
- * 4-byte flag per batch of candidates). */
+ * as that rule would.  Synchronous (one host read of
+ * two 4-byte flags per batch of candidates). */
 int solve_projection(const float* f0, const float* mean, const float* U, int K, const float* y,
                      const pcas_vol* vol, const pcas_cb* cb, const double* w_init,
                      const pcas_params* params, double* w_out, pcas_stats* stats, void* ws,
@@ -244,6 +245,8 @@ int pcas_solver_destroy(pcas_solver solver);
  * Solves staged at exactly that angle and those offsets (pcas_solver_solve,
  * runs, batches) then read these weights instead of recomputing them; the
  * sums keep their order, so results are bitwise those of the uncached solver.
+ * (Where an eighth of the voxels or more have a non-zero warp Jacobian, as in a
+ * CT with texture, the gradient walks voxel columns instead, cached or not.)
  * pcas_solver_fixed_view_bytes: device bytes of the cache for angle_rad (0 if
  *   the solver or the view is invalid, or a detector side exceeds 32767
  *   pixels).  Counts on the device on `stream`; synchronous.
