@@ -156,8 +156,8 @@ k_warp_dvf(const T* __restrict__ f0, const float* __restrict__ dvf, Grid g, floa
 // The halo copy of the reference CT (see tri_halo), halo included: a warp per
 // row, 128 values in flight.  With f0m (zeroed by the caller) it marks the
 // bricks whose taps include a non-zero voxel (see Occ): voxel i is a tap of the
-// cells of bricks i >> 3 and (i + 1) >> 3 along each axis; one lane marks the
-// span of the non-zero voxels among 32 of a row.  skip (may be null): when it
+// cells of bricks i >> 3 and (i + 1) >> 3 along each axis; the lanes mark the
+// span of the non-zero voxels among 32 of a row, a brick each.  skip (may be null): when it
 // holds a non-zero value the copy is current and the kernel returns at once.
 // Bound by HBM: 256x256x100 48 us (interior alone, a block per row, after a
 // memset of 6 us) -> 14 us, 512x512x160 from bfloat16 199 + 26 -> 80 us.
@@ -190,11 +190,11 @@ k_fill_f0h(const T* __restrict__ f0, Grid g, float* __restrict__ f0h, unsigned c
 #pragma unroll
             for (int e = 0; e < 4; e++) {
                 const unsigned live = __ballot_sync(0xffffffffu, v[e] != 0.0f);
-                if (lane != 0 || live == 0) continue;
+                if (live == 0) continue;
+                // the bricks of the span, one per lane: 5 at most along x, 2 along y and z
                 const int i = x0 + 32 * e - F0_HALO, lo = i + __ffs((int)live) - 1, hi = i + 31 - __clz((int)live);
-                for (int bz = k >> 3; bz <= (k + 1) >> 3; bz++)
-                    for (int by = j >> 3; by <= (j + 1) >> 3; by++)
-                        for (int bx = lo >> 3; bx <= (hi + 1) >> 3; bx++) f0m[(bz * nby + by) * nbx + bx] = 1;
+                const int bx = (lo >> 3) + (lane & 7), by = (j >> 3) + ((lane >> 3) & 1), bz = (k >> 3) + (lane >> 4);
+                if (bx <= (hi + 1) >> 3 && by <= (j + 1) >> 3 && bz <= (k + 1) >> 3) f0m[(bz * nby + by) * nbx + bx] = 1;
             }
         }
     }
