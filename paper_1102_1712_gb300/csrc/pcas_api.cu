@@ -478,9 +478,11 @@ int check_finite(const double* v, int n, const char* name) {
 
 // The start of an evaluation or solve, in one launch: the solver state, the
 // view, the reference CT's bricks and the halos of the solver volumes (whose
-// interior the warps write whole).  Zeroing the volumes whole took 20 us at
-// 256x256x100 and 110 us at 512x512x160; the halos, the state and the view
-// (separate launches and copies before) take 5 and 12.
+// interior the warps write whole).  Before, two memsets (cost_grad zeroed 115 MB
+// of volumes and halo copy at 256x256x100, 708 MB at 512x512x160), a launch for
+// the state and a copy for the view; this launch takes 6 and 10 us (3 at 61x53x29),
+// and with the halo copy (k_fill_f0h) cost_grad went 690 -> 644 us, 3.97 -> 3.75
+// ms and 120 -> 110 us.
 struct HaloRows {             // a volume of rows pitch floats long: interior [lo, hi) in rows
     float* p;                 // 2 <= j < ny + 2, 2 <= k < nz + 2 of pny x pnz
     int pitch, lo, hi;

@@ -159,8 +159,10 @@ k_warp_dvf(const T* __restrict__ f0, const float* __restrict__ dvf, Grid g, floa
 // cells of bricks i >> 3 and (i + 1) >> 3 along each axis; the lanes mark the
 // span of the non-zero voxels among 32 of a row, a brick each.  skip (may be null): when it
 // holds a non-zero value the copy is current and the kernel returns at once.
-// Bound by HBM: 256x256x100 48 us (interior alone, a block per row, after a
-// memset of 6 us) -> 14 us, 512x512x160 from bfloat16 199 + 26 -> 80 us.
+// Bound by latency at 256x256x100 (26 MB from HBM, 29 MB left in L2) and by HBM
+// beyond: 48 us (interior alone, a block per row, after a memset of 6 us) -> 37
+// with a warp per row -> 22 with the marks spread over the lanes; 512x512x160
+// from bfloat16 199 + 26 -> 76 us.
 template <typename T>
 __global__ void __launch_bounds__(kWarpThreads)
 k_fill_f0h(const T* __restrict__ f0, Grid g, float* __restrict__ f0h, unsigned char* __restrict__ f0m,
