@@ -80,47 +80,70 @@ k_pca_dvf(const T* __restrict__ mean, const T* __restrict__ U, int K, WSrc ws, l
     }
 }
 
-// Warp by an explicit DVF (public warp_volume), dense out: kDvfVPT voxels of a
-// row per thread, blockDim.x apart, their DVF loads issued together (the DVF
-// streams past the caches, which the gathers need), no index division.
-// Bound by L1 (neighbouring voxels' taps lie in many rows where the field is
-// steep): 512x512x160 281 us with an index division and bounds tests a voxel,
-// 245 here (3.4 TB/s); 256x256x100 with the DVF's synthesis 98 -> 89 us.  One
-// voxel a thread 263, four 244 (256x256x100: 92 and 94).
-constexpr int kDvfVPT = 2;
-template <typename T>
-__global__ void __launch_bounds__(kWarpThreads, 6)
-k_warp_dvf(const T* __restrict__ f0, const float* __restrict__ dvf, Grid g, float* __restrict__ f) {
-    const int j = blockIdx.y, k = blockIdx.z;
-    const long N = (long)g.nx * g.ny * g.nz;
-    const long row = ((long)k * g.ny + j) * g.nx;
-    const int i0 = blockIdx.x * blockDim.x * kDvfVPT + threadIdx.x;
-    float x[kDvfVPT][3];
+// n / d for n < 2^31 as one product and a shift (T. Granlund and P. Montgomery,
+// "Division by invariant integers using multiplication", 1994): with l the
+// ceiling of log2 d and m = floor(2^(31 + l) / d) + 1 < 2^32, m d exceeds
+// 2^(31 + l) by at most 2^l, so that n m / 2^(31 + l) exceeds n / d by less than 1 / d.
+struct FastDiv {
+    unsigned m;
+    int shift;
+};
+inline FastDiv fast_div(unsigned d) {
+    int l = 0;
+    while ((1ull << l) < d) l++;
+    return {(unsigned)((1ull << (31 + l)) / d + 1), 31 + l};
+}
+__device__ __forceinline__ unsigned div_by(FastDiv f, unsigned n) {
+    return (unsigned)(((unsigned long long)n * f.m) >> f.shift);
+}
+
+// Warp by an explicit DVF (public warp_volume), dense out: VPT voxels per thread,
+// blockDim.x apart in the flat order, so that rows of any length fill the
+// blocks; their DVF loads go out together and past the caches, which the
+// gathers need.  With VPT = 2 and every cell of the thread in the grid all
+// sixteen taps are in flight at once, without tests.
+// Bound by L1 beyond the caches' reach (neighbouring voxels' taps lie in many
+// rows where the field is steep) and by latency below it.  One voxel a thread
+// and eight blocks per SM, or two and six (us a launch):
+//   96x90x48 3.9 / 5.0, 149x131x67 8.4 / 9.5, 224x200x100 23.4 / 23.8,
+//   256x256x100 34.8 / 34.3, 400x380x120 107 / 103, 512x512x160 238 / 231 (3.6 TB/s)
+// hence two from kDvfPairs voxels on.  Blocks within a row, two voxels a thread,
+// leave lanes idle in rows that are no multiple of 64: 6.1 us at 96x90x48, 130
+// at 400x380x120.
+constexpr long kDvfPairs = 6000000;
+template <int VPT, typename T>
+__global__ void __launch_bounds__(kWarpThreads, VPT == 1 ? 8 : 6)
+k_warp_dvf(const T* __restrict__ f0, const float* __restrict__ dvf, Grid g, FastDiv by_nx, FastDiv by_ny,
+           float* __restrict__ f) {
+    const unsigned N = (unsigned)g.nx * g.ny * g.nz;             // < 2^31
+    unsigned n[VPT];
+    n[0] = blockIdx.x * (kWarpThreads * VPT) + threadIdx.x;
+    if (n[0] >= N) return;
+    float x[VPT][3];
 #pragma unroll
-    for (int e = 0; e < kDvfVPT; e++) {
-        const int i = i0 + e * blockDim.x;
+    for (int e = 0; e < VPT; e++) {
+        n[e] = n[0] + e * kWarpThreads < N ? n[0] + e * kWarpThreads : n[0];     // past the volume: the first once more
 #pragma unroll
-        for (int c = 0; c < 3; c++) x[e][c] = i < g.nx ? __ldcs(dvf + c * N + row + i) : 0.0f;
+        for (int c = 0; c < 3; c++) x[e][c] = __ldcs(dvf + (long)c * N + n[e]);
     }
     // the usual case, every cell of the thread's voxels in the grid: all their
     // taps in flight together, no tests
     const int sy = g.nx, sz = g.nx * g.ny;
-    float z[kDvfVPT][3];
-    int at[kDvfVPT];
     bool inner = true;
 #pragma unroll
-    for (int e = 0; e < kDvfVPT; e++) {
-        const int i = min(i0 + e * (int)blockDim.x, g.nx - 1);               // (past the row: its last voxel's place)
-        x[e][0] = fmaf(x[e][0], g.inv_sx, (float)i);
-        x[e][1] = fmaf(x[e][1], g.inv_sy, (float)j);
-        x[e][2] = fmaf(x[e][2], g.inv_sz, (float)k);
+    for (int e = 0; e < VPT; e++) {
+        const unsigned r = div_by(by_nx, n[e]), k = div_by(by_ny, r);
+        x[e][0] = fmaf(x[e][0], g.inv_sx, (float)(int)(n[e] - r * g.nx));
+        x[e][1] = fmaf(x[e][1], g.inv_sy, (float)(int)(r - k * g.ny));
+        x[e][2] = fmaf(x[e][2], g.inv_sz, (float)(int)k);
         inner = inner && x[e][0] >= 0.0f && x[e][1] >= 0.0f && x[e][2] >= 0.0f && x[e][0] < (float)(g.nx - 1) &&
                 x[e][1] < (float)(g.ny - 1) && x[e][2] < (float)(g.nz - 1);
     }
-    if (inner) {
-        float v[kDvfVPT][8];
+    if (VPT > 1 && inner) {
+        float z[VPT][3], v[VPT][8];
+        int at[VPT];
 #pragma unroll
-        for (int e = 0; e < kDvfVPT; e++) {
+        for (int e = 0; e < VPT; e++) {
             int lx, ly, lz;
             z[e][0] = x[e][0] - floor_int(x[e][0], lx);
             z[e][1] = x[e][1] - floor_int(x[e][1], ly);
@@ -128,25 +151,21 @@ k_warp_dvf(const T* __restrict__ f0, const float* __restrict__ dvf, Grid g, floa
             at[e] = lz * sz + ly * sy + lx;
         }
 #pragma unroll
-        for (int e = 0; e < kDvfVPT; e++)
+        for (int e = 0; e < VPT; e++)
 #pragma unroll
             for (int t = 0; t < 8; t++)
                 v[e][t] = ldg_f(f0 + at[e] + ((t & 1) + ((t & 2) ? sy : 0) + ((t & 4) ? sz : 0)));
 #pragma unroll
-        for (int e = 0; e < kDvfVPT; e++) {
-            const int i = i0 + e * blockDim.x;
+        for (int e = 0; e < VPT; e++) {
             const float c00 = fmaf(z[e][0], v[e][1] - v[e][0], v[e][0]), c10 = fmaf(z[e][0], v[e][3] - v[e][2], v[e][2]);
             const float c01 = fmaf(z[e][0], v[e][5] - v[e][4], v[e][4]), c11 = fmaf(z[e][0], v[e][7] - v[e][6], v[e][6]);
             const float c0 = fmaf(z[e][1], c10 - c00, c00), c1 = fmaf(z[e][1], c11 - c01, c01);
-            if (i < g.nx) __stcs(f + row + i, fmaf(z[e][2], c1 - c0, c0));
+            __stcs(f + n[e], fmaf(z[e][2], c1 - c0, c0));
         }
         return;
     }
 #pragma unroll
-    for (int e = 0; e < kDvfVPT; e++) {
-        const int i = i0 + e * blockDim.x;
-        if (i < g.nx) __stcs(f + row + i, tri_dense(f0, g, x[e][0], x[e][1], x[e][2]));
-    }
+    for (int e = 0; e < VPT; e++) __stcs(f + n[e], tri_dense(f0, g, x[e][0], x[e][1], x[e][2]));
 }
 
 // Thread layout of the solver warps: blockIdx.z = k, blockIdx.y = j and
@@ -469,9 +488,14 @@ cudaError_t launch_pca_dvf(const void* mean, const void* U, int dt, int K, const
 }
 
 cudaError_t launch_warp_dvf(const void* f0, int dt, const float* dvf, Grid g, float* f, cudaStream_t s) {
-    const RowLaunch L = row_launch(g, kDvfVPT);
-    PCAS_DT_DISPATCH(dt, (k_warp_dvf<T><<<L.grid, L.threads, 0, s>>>(static_cast<const T*>(f0), dvf, g, f),
-                          cudaGetLastError()))
+    const long N = (long)g.nx * g.ny * g.nz;
+    const FastDiv by_nx = fast_div(g.nx), by_ny = fast_div(g.ny);
+    if (N < kDvfPairs) {
+        PCAS_DT_DISPATCH(dt, (k_warp_dvf<1, T><<<blocks_for(N), kWarpThreads, 0, s>>>(
+                                  static_cast<const T*>(f0), dvf, g, by_nx, by_ny, f), cudaGetLastError()))
+    }
+    PCAS_DT_DISPATCH(dt, (k_warp_dvf<2, T><<<blocks_for((N + 1) / 2), kWarpThreads, 0, s>>>(
+                              static_cast<const T*>(f0), dvf, g, by_nx, by_ny, f), cudaGetLastError()))
 }
 
 cudaError_t launch_fill_f0h(const void* f0, int dt, Grid g, float* f0h, unsigned char* f0m, const int* skip,
