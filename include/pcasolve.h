@@ -193,7 +193,9 @@ int solve_projection(const float* f0, const float* mean, const float* U, int K, 
  * iterate y <- -x(c_ref + y) from y = 0 (x trilinear in mm, zero outside the
  * grid) until the update is below tol_mm or max_iter is reached; c = c_ref + y.
  * mean, U: device; w (K), c_ref, c_out: host.  Synchronous.  Returns
- * PCAS_NOT_CONVERGED (with c_out set) if the cap was reached. */
+ * PCAS_NOT_CONVERGED (with c_out set) if the cap was reached.  A component
+ * whose update is not a number counts as unchanged: where the DVF at the
+ * iterate is NaN the iteration ends (PCAS_OK) with NaN in those of c_out. */
 int localize_tumor(const float* mean, const float* U, int K, const double* w,
                    const pcas_vol* vol, const double c_ref[3], int max_iter, double tol_mm,
                    double c_out[3], void* stream);

@@ -380,7 +380,9 @@ int gather_blocks(const Tune& T) {
 // A chain of dependent FP64 operations, at a 64th of FP32's rate: eight lanes
 // with a tap each, their weights and three sums over lanes took 45 us for 50
 // iterations and the whole call 67 us; now the call takes 46.
-// Lane 0 writes out[0..2] = c and out[3] = 1 if it converged (else 0).
+// Lane 0 writes out[0..2] = c and out[3] = 1 if it converged (else 0).  A component
+// whose update is not a number does not count as a change, so that a field of NaN
+// at the iterate ends the iteration, with NaN in c.
 template <typename T>
 __device__ void localize_warp(const T* __restrict__ mean, const T* __restrict__ U, int K, const Grid& g,
                               const double* w, double ox, double oy, double oz, double isx, double isy,
@@ -430,7 +432,7 @@ __device__ void localize_warp(const T* __restrict__ mean, const T* __restrict__ 
                 if (wt != 0.0) x += wt * v[e];
             }
         }
-        const double change = fabs(-x - y);
+        const double change = fmax(fabs(-x - y), 0.0);     // 0 where the field is not a number
         y = -x;
         if (__all_sync(0xffffffffu, change < tol)) { converged = 1; break; }
     }
