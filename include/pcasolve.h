@@ -247,8 +247,9 @@ int pcas_solver_destroy(pcas_solver solver);
  * Solves staged at exactly that angle and those offsets (pcas_solver_solve,
  * runs, batches) then read these weights instead of recomputing them; the
  * sums keep their order, so results are bitwise those of the uncached solver.
- * (Where an eighth of the voxels or more have a non-zero warp Jacobian, as in a
- * CT with texture, the gradient walks voxel columns instead, cached or not.)
+ * (Where the voxels with a non-zero warp Jacobian are many and close together,
+ * as in a CT with texture, the gradient walks voxel columns instead, cached or
+ * not.)
  * pcas_solver_fixed_view_bytes: device bytes of the cache for angle_rad (0 if
  *   the solver or the view is invalid, or a detector side exceeds 32767
  *   pixels).  Counts on the device on `stream`; synchronous.
