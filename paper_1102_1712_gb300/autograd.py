@@ -55,8 +55,8 @@ class CostFunction(torch.autograd.Function):
                                         prob.step, want_grad=True, want_grad_f0=need_f0, ws=prob.ws)
         gw = ((torch.from_numpy(np.asarray(G)).to(w.dtype) * gJ.detach().to("cpu", w.dtype)).to(w.device)
               if need_w else None)
-        gf0 = ((dJdf0 * gJ.to(dJdf0.device, torch.float32, non_blocking=True)).view_as(f0)
-               if need_f0 else None)
+        # J lives on the host, and so does gJ: a number to the product's kernel, read here
+        gf0 = (dJdf0 * gJ.to("cpu", torch.float32)).view_as(f0) if need_f0 else None
         return gw, gf0, None
 
 
