@@ -1103,15 +1103,17 @@ int pcas_autotune(const void* f0, const void* mean, const void* U, int dtype, in
         if (tt[1 - cur] < keep * tt[cur]) best.swap[b] = (unsigned char)(1 - cur);
     }
     // 2. per angle bin, the patch width and chunk of the batch projector (the
-    //    same rule: the incumbent, else the first within the margin)
+    //    same rule: the incumbent, else the first within the margin); on detectors
+    //    whose batch stages nothing (drr_splits) the chunk stays what it is
     for (int b = 0; b < NBIN && rc == PCAS_OK; b++) {
         if (!ok_bin[b]) continue;
-        const int chunks[3] = {12, 16, 24};
         double bestt = 0.0, inct = -1.0, tc[3][3];
         const int ilw = best.lw4[b], ich = best.chunk4[b];
+        const bool splits = drr_splits(cb->nu, cb->nv, TRIAL_BATCH);
+        const int chunks[3] = {splits ? ich : 12, 16, 24}, nchunks = splits ? 1 : 3;
         bool any = false;
         for (int lw = 2; lw <= 4 && rc == PCAS_OK; lw++) {
-            for (int c = 0; c < 3 && rc == PCAS_OK; c++) {
+            for (int c = 0; c < nchunks && rc == PCAS_OK; c++) {
                 tc[lw - 2][c] = -1.0;
                 Tune X = best;
                 X.lw4[b] = (unsigned char)lw;
@@ -1128,7 +1130,7 @@ int pcas_autotune(const void* f0, const void* mean, const void* U, int dtype, in
         if (rc != PCAS_OK || !any || (inct > 0.0 && bestt > keep * inct)) continue;
         bool set = false;
         for (int lw = 2; lw <= 4 && !set; lw++)
-            for (int c = 0; c < 3 && !set; c++)
+            for (int c = 0; c < nchunks && !set; c++)
                 if (tc[lw - 2][c] > 0.0 && keep * tc[lw - 2][c] <= bestt) {
                     best.lw4[b] = (unsigned char)lw;
                     best.chunk4[b] = (unsigned char)chunks[c];
