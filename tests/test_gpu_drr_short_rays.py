@@ -1,9 +1,10 @@
-"""drr_forward where rays are short and many: values on both sides of the line
-between four and eight warps a patch against the FP64 oracle (1e-4 of the
-maximum, as in the other DRR tests), and the time of 48 voxels across against 128
-on the same large detector.  The latter has 2.7 times the samples; what both have
-alike is a ray's set-up, once a warp.  Measured: 0.44 with four warps a patch,
-0.49 with eight, which is more than one thread a ray takes; the line is between."""
+"""drr_forward where rays are short and many: values on both sides of the lines
+between a thread per ray, four and eight warps a patch against the FP64 oracle
+(1e-4 of the maximum, as in the other DRR tests), and two times on the same large
+detector, of what have alike a ray's set-up, once a warp.  48 voxels across
+against 128, 2.7 times the samples: 0.44 with four warps a patch, 0.49 with eight,
+which is more than one thread a ray takes; the line is between.  8 voxels across
+against 48: 0.47 with a thread per ray, 0.71 with eight warps a patch."""
 import numpy as np
 import pytest
 
@@ -54,6 +55,6 @@ def test_time_of_short_rays(P):
         b.synchronize()
         return a.elapsed_time(b)
 
-    short, long = problem((48, 44, 24)), problem((128, 128, 64))
-    t = [(ms(short), ms(long)) for _ in range(10)][2:]
-    assert min(x[0] for x in t) <= 0.465 * min(x[1] for x in t)
+    q = [problem(n) for n in ((8, 8, 8), (48, 44, 24), (128, 128, 64))]
+    t = np.min([[ms(p) for p in q] for _ in range(10)][2:], axis=0)
+    assert t[1] <= 0.465 * t[2] and t[0] <= 0.59 * t[1], t
