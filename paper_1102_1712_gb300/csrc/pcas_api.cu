@@ -148,6 +148,7 @@ int make_view(const pcas_vol* vol, const pcas_cb* cb, double step, View* V) {
     const double ew[3] = {-sa, ca, 0.0}, eu[3] = {ca, sa, 0.0}, ev[3] = {0.0, 0.0, 1.0};
     const double o[3] = {vol->ox, vol->oy, vol->oz}, s[3] = {vol->sx, vol->sy, vol->sz};
     const int n[3] = {vol->nx, vol->ny, vol->nz};
+    double nearest = 1e300;
     for (int corner = 0; corner < 8; corner++) {   // whole support box ahead of the source
         double dot = 0;
         for (int c = 0; c < 3; c++) {
@@ -156,6 +157,7 @@ int make_view(const pcas_vol* vol, const pcas_cb* cb, double step, View* V) {
         }
         if (!(dot > 0))
             return fail(PCAS_ERR_INVALID_ARG, "the volume must lie entirely in front of the source");
+        nearest = fmin(nearest, dot);
     }
     if ((double)cb->sdd * 4.0 > 1e30) return fail(PCAS_ERR_INVALID_ARG, "sdd too large");
     // sample indices i = t/step must stay far inside the int range
@@ -181,6 +183,9 @@ int make_view(const pcas_vol* vol, const pcas_cb* cb, double step, View* V) {
     V->step = (float)step;
     // symmetric to within the rounding of the float geometry
     V->zsym = fabs(cb->off_v) <= 1e-9 * cb->dv && fabs(vol->oz + 0.5 * (vol->nz - 1) * vol->sz) <= 1e-9 * vol->sz;
+    const double wide = fmax(s[0], s[1]), high = fmax(fabs(o[2] - s[2]), fabs(o[2] + n[2] * s[2]));
+    V->columns = columns_suit(make_grid(vol), V->zsym != 0, 2.0 * M_SQRT2 * wide / step,
+                              2.4 * wide * (high / nearest) / s[2] + 1.0);
     V->swap = 0;                            // launch shapes: set_layouts
     V->lw1 = V->lw4 = 3;
     V->chunk1 = 0;
@@ -887,7 +892,7 @@ int cost_grad_f0(const float* f0, const float* mean, const float* U, int K, cons
                     launch_adjoint_grad(W.rayt, g, W.view, W.f0h, occ_of(W, T).f0m, mean, U, DT_F32, K, 0, W.st,
                                         W.part_adj, W.adj, T.vt, gather_blocks(T), 0ull, 0, nullptr, GradRun{false, -1}, s));
     if (dJdf0)
-        PCAS_LAUNCH(PCAS_K_GRAD_F0, s, launch_grad_f0(W.rayt, g, W.view, mean, U, K, W.st, z, zmax, acc, dJdf0, s));
+        PCAS_LAUNCH(PCAS_K_GRAD_F0, s, launch_grad_f0(W.rayt, g, W.view, V.columns, mean, U, K, W.st, z, zmax, acc, dJdf0, s));
     SolveState h;
     PCAS_CUDA(cudaMemcpyAsync(&h, W.st, sizeof(h), cudaMemcpyDeviceToHost, s));
     PCAS_CUDA(cudaStreamSynchronize(s));
