@@ -1,7 +1,8 @@
 """warp_volume on rows of any length: values against the FP64 oracle on both
 sides of the size from which a thread takes two voxels (an odd voxel count
 among them, so that the last thread has one), 5e-5 of the maximum as in the
-other warp tests; and the time per voxel, which must not depend on whether the
+other warp tests, whose extents are below 256, and more in proportion to larger
+ones (a position's rounding); and the time per voxel, which must not depend on whether the
 rows are a multiple of a warp: 400x360x100 against 384x360x100 has the same
 work per voxel, so the ratio is 1 but for the lanes and tests that a launch
 wastes on its rows' ends (1.25 with blocks that end with the row); the line is
@@ -35,7 +36,7 @@ def test_values(P, dims):
     dvf = g.uniform(-6.0, 6.0, 3 * f0.size).astype(np.float32)
     got = P.warp_volume(torch.from_numpy(f0).cuda(), torch.from_numpy(dvf).cuda(), vol).cpu().numpy()
     ref = O.warp_volume(f0.reshape(dims[::-1]), dvf.reshape(3, -1), vol)
-    assert np.abs(got - ref.ravel()).max() <= 5e-5 * f0.max()
+    assert np.abs(got - ref.ravel()).max() <= 5e-5 * max(1.0, max(dims) / 256) * f0.max()
 
 
 def test_time_per_voxel_of_ragged_rows(P):
