@@ -220,9 +220,9 @@ Layout layout(const pcas_vol* vol, const pcas_cb* cb, int K) {
     L.state = off; off += align256(sizeof(SolveState));
     L.view = off; off += align256(sizeof(View));
     L.f0h = off; off += align256((size_t)f0h_count(vol->nx, vol->ny, vol->nz) * sizeof(float));  // f0, halo 3
-    L.f0m = off; off += align256((size_t)f0b_count(vol->nx, vol->ny, vol->nz));     // its bricks (zeroed with it)
-    L.fpad = off; off += align256(npad * sizeof(float));                 // f(w), zero halo
-    L.fpair = off; off += align256(npad * sizeof(float2));               // f(w) as x pairs (the L1 march)
+    L.f0m = off; off += align256((size_t)f0b_count(vol->nx, vol->ny, vol->nz));     // its bricks
+    L.fpad = off; off += align256(npad * sizeof(float));                 // candidate 4, zero halo
+    L.fpair = off; off += align256(npad * sizeof(float2));               // f(w) as x pairs, zero halo
     L.fpad4 = off; off += align256(npad * sizeof(float4));               // candidates 0-3 (4 in fpad)
     L.occ = off; off += align256((size_t)occ_count(vol->nx, vol->ny, vol->nz) * sizeof(unsigned int));
     L.pbuf = off; off += align256((size_t)NBUF * M * sizeof(float));     // projection ring
@@ -290,17 +290,13 @@ inline Occ occ_of(const Ws& W, const Tune& T) {
     return Occ{T.skip ? W.occ : nullptr, &W.st->occ_gen, T.skip ? W.f0m : nullptr};
 }
 
-// Where the one-volume warp writes f(w): its x-pair copy, which the one-volume
-// projector reads (through L1, or staged chunk by chunk).
-inline float2* pair_of(const Ws& W, const Tune&) { return W.fpair; }
-
 // The first evaluation's warp of a solve at the staged w (st->w), fused with
 // the Jacobian pass of the gradient at that w (launch_warp_jac): the next
 // launch_adjoint_grad with T.vt skips its own.
 inline cudaError_t first_warp(const Ws& W, const Tune& T, const Grid& g, const void* mean, const void* U, int dt,
                               int K, cudaStream_t s) {
     const Occ oc = occ_of(W, T);
-    const JacWarp jw{W.view, W.fpad, pair_of(W, T), W.st->box[0], oc};
+    const JacWarp jw{W.view, W.fpair, W.st->box[0], oc};
     return launch_warp_jac(g, W.f0h, oc.f0m, mean, U, dt, K, W.st, W.adj, T.vt, jw, s);
 }
 
@@ -485,11 +481,10 @@ int check_finite(const double* v, int n, const char* name) {
 
 // The start of an evaluation or solve, in one launch: the solver state, the
 // view, the reference CT's bricks and the halos of the solver volumes (whose
-// interior the warps write whole).  Before, two memsets (cost_grad zeroed 115 MB
-// of volumes and halo copy at 256x256x100, 708 MB at 512x512x160), a launch for
-// the state and a copy for the view; this launch takes 6 and 10 us (3 at 61x53x29),
-// and with the halo copy (k_fill_f0h) cost_grad went 690 -> 644 us, 3.97 -> 3.75
-// ms and 120 -> 110 us.
+// interior the warps write whole): 6 us at 256x256x100, 10 at 512x512x160, 3 at
+// 61x53x29.  Memsets of whole volumes and halo copy (115 MB, 708 MB), a launch for
+// the state and a copy for the view cost cost_grad 690 us where it takes 657, 3.97
+// ms for 3.81, 120 us for 110.
 struct HaloRows {             // a volume of rows pitch floats long: interior [lo, hi) in rows
     float* p;                 // 2 <= j < ny + 2, 2 <= k < nz + 2 of pny x pnz
     int pitch, lo, hi;
@@ -881,8 +876,8 @@ int cost_grad_f0(const float* f0, const float* mean, const float* U, int K, cons
     if (dJdw || !warp_pca_fits(mean, U, DT_F32, g))
         PCAS_LAUNCH(PCAS_K_WARP_PCA, s, first_warp(W, T, g, mean, U, DT_F32, K, s));
     else
-        PCAS_LAUNCH(PCAS_K_WARP_PCA, s, launch_warp_pca(W.f0h, mean, U, DT_F32, K, wsrc, g, W.view, W.fpad,
-                                                        pair_of(W, T), W.st->box[0], occ_of(W, T), s));
+        PCAS_LAUNCH(PCAS_K_WARP_PCA, s, launch_warp_pca(W.f0h, mean, U, DT_F32, K, wsrc, g, W.view, W.fpair,
+                                                        W.st->box[0], occ_of(W, T), s));
     PCAS_LAUNCH(PCAS_K_DRR_SOLVER, s,
                 launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, 0, W.st, W.part_drr, W.part_adj,
                                   T, 0ull, 0, occ_of(W, T), s));

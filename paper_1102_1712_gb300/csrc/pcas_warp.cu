@@ -178,10 +178,9 @@ k_warp_dvf(const T* __restrict__ f0, const float* __restrict__ dvf, Grid g, Fast
 // cells of bricks i >> 3 and (i + 1) >> 3 along each axis; the lanes mark the
 // span of the non-zero voxels among 32 of a row, a brick each.  skip (may be null): when it
 // holds a non-zero value the copy is current and the kernel returns at once.
-// Bound by latency at 256x256x100 (26 MB from HBM, 29 MB left in L2) and by HBM
-// beyond: 48 us (interior alone, a block per row, after a memset of 6 us) -> 37
-// with a warp per row -> 22 with the marks spread over the lanes; 512x512x160
-// from bfloat16 199 + 26 -> 76 us.
+// Bound by latency at 256x256x100 (26 MB from HBM, 29 MB left in L2; 22 us, 37 with
+// one lane marking the bricks, 48 and a memset of 6 with a block per row and the
+// interior alone) and by HBM beyond (512x512x160 from bfloat16 76 us, 199 and 26).
 template <typename T>
 __global__ void __launch_bounds__(kWarpThreads)
 k_fill_f0h(const T* __restrict__ f0, Grid g, float* __restrict__ f0h, unsigned char* __restrict__ f0m,
@@ -221,11 +220,10 @@ k_fill_f0h(const T* __restrict__ f0, Grid g, float* __restrict__ f0h, unsigned c
     }
 }
 
-// Fused DVF synthesis + warp into the zero-halo layout used by the solver
-// (fpad), or into its x-pair copy (fpair not null: each voxel stored as the
-// first value of its own pair and the second of the pair before it; the
-// pairs' halo values stay the zeros the caller wrote); marks the occupancy
-// bricks of its non-zero voxels.
+// Fused DVF synthesis + warp into the zero-halo layout used by the solver, as x
+// pairs (each voxel stored as the first value of its own pair and the second of
+// the pair before it; the pairs' halo values stay the zeros the caller wrote);
+// marks the occupancy bricks of its non-zero voxels.
 // 4 voxels per thread along x (nx % 4 == 0, 16-byte aligned model; other rows
 // go through launch_warp_jac, whose coalesced single loads take half the time
 // of one voxel a thread here: 149x131x67, K = 2, 46 -> 24 us).
@@ -233,7 +231,7 @@ template <typename T>
 __global__ void __launch_bounds__(kWarpThreads)
 k_warp_pca(const float* __restrict__ f0h, const T* __restrict__ mean,
            const T* __restrict__ U, int K, WSrc ws, Grid g, const View* __restrict__ Vp,
-           float* __restrict__ fpad, float2* __restrict__ fpair, int* __restrict__ box_out, Occ occ) {
+           float2* __restrict__ fpair, int* __restrict__ box_out, Occ occ) {
     if (ws.phase && *ws.phase >= PH_STOP) return;
     const int swp = Vp ? Vp->swap : 0;
     const Pad pd = solver_pad(g.nx, g.ny, g.nz, swp);
@@ -273,27 +271,20 @@ k_warp_pca(const float* __restrict__ f0h, const T* __restrict__ mean,
             if (swp) occ_mark(oc.m, oc.gen, oc.nbx, oc.nby, j, j, i + e0, i + e1, k);
             else occ_mark(oc.m, oc.gen, oc.nbx, oc.nby, i + e0, i + e1, j, j, k);
         }
-        if (fpair) {                    // voxel d is .x of pair d and .y of pair d - 1
-            float* p = reinterpret_cast<float*>(fpair);
-            if (swp) {
+        float* p = reinterpret_cast<float*>(fpair);         // voxel d is .x of pair d and .y of pair d - 1
+        if (swp) {
 #pragma unroll
-                for (int e = 0; e < 4; e++) {
-                    const long d = pad_index(pd, j, i + e, k);
-                    p[2 * d - 1] = o[e];
-                    p[2 * d] = o[e];
-                }
-            } else {                    // d a multiple of 4: floats 2d - 1 ... 2d + 6
-                const long d = pad_index(pd, i, j, k);
-                p[2 * d - 1] = o[0];
-                *reinterpret_cast<float4*>(p + 2 * d) = make_float4(o[0], o[1], o[1], o[2]);
-                *reinterpret_cast<float2*>(p + 2 * d + 4) = make_float2(o[2], o[3]);
-                p[2 * d + 6] = o[3];
+            for (int e = 0; e < 4; e++) {
+                const long d = pad_index(pd, j, i + e, k);
+                p[2 * d - 1] = o[e];
+                p[2 * d] = o[e];
             }
-        } else if (swp) {
-#pragma unroll
-            for (int e = 0; e < 4; e++) fpad[pad_index(pd, j, i + e, k)] = o[e];
-        } else {
-            *reinterpret_cast<float4*>(fpad + pad_index(pd, i, j, k)) = make_float4(o[0], o[1], o[2], o[3]);
+        } else {                        // d a multiple of 4: floats 2d - 1 ... 2d + 6
+            const long d = pad_index(pd, i, j, k);
+            p[2 * d - 1] = o[0];
+            *reinterpret_cast<float4*>(p + 2 * d) = make_float4(o[0], o[1], o[1], o[2]);
+            *reinterpret_cast<float2*>(p + 2 * d + 4) = make_float2(o[2], o[3]);
+            p[2 * d + 6] = o[3];
         }
     }
     box_reduce(b, box_out);
@@ -447,13 +438,13 @@ cudaError_t pca_dvf_t(const void* mean, const void* U, int K, const float* w, Gr
 
 template <typename T>
 cudaError_t warp_pca_t(const float* f, const void* mean, const void* U, int K, WSrc w, Grid g,
-                       const View* Vd, float* fpad, float2* fpair, int* box, Occ oc, cudaStream_t s) {
+                       const View* Vd, float2* fpair, int* box, Occ oc, cudaStream_t s) {
     const unsigned a = sizeof(T) * 4;
-    if (g.nx % 4 || !aligned(mean, a) || !aligned(U, a) || !aligned(fpad, 16) || !aligned(fpair, 16))
+    if (g.nx % 4 || !aligned(mean, a) || !aligned(U, a) || !aligned(fpair, 16))
         return cudaErrorInvalidValue;       // warp_pca_fits
     const RowLaunch L = row_launch(g, 4);
     k_warp_pca<T><<<L.grid, L.threads, 0, s>>>(f, static_cast<const T*>(mean), static_cast<const T*>(U), K, w, g, Vd,
-                                               fpad, fpair, box, oc);
+                                               fpair, box, oc);
     return cudaGetLastError();
 }
 
@@ -512,8 +503,8 @@ bool warp_pca_fits(const void* mean, const void* U, int dt, const Grid& g) {
 }
 
 cudaError_t launch_warp_pca(const float* f0, const void* mean, const void* U, int dt, int K, WSrc w,
-                            Grid g, const View* Vd, float* fpad, float2* fpair, int* box, Occ oc, cudaStream_t s) {
-    PCAS_DT_DISPATCH(dt, (warp_pca_t<T>(f0, mean, U, K, w, g, Vd, fpad, fpair, box, oc, s)))
+                            Grid g, const View* Vd, float2* fpair, int* box, Occ oc, cudaStream_t s) {
+    PCAS_DT_DISPATCH(dt, (warp_pca_t<T>(f0, mean, U, K, w, g, Vd, fpair, box, oc, s)))
 }
 
 cudaError_t launch_warp_batch(const float* f0, const void* mean, const void* U, int dt, int K,
