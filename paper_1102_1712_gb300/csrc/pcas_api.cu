@@ -765,12 +765,18 @@ int drr_siddon(const float* f, const pcas_vol* vol, const pcas_cb* cb, float* p,
     const double ew[3] = {-sa, ca, 0.0}, eu[3] = {ca, sa, 0.0}, ev[3] = {0.0, 0.0, 1.0};
     for (int c = 0; c < 3; c++) { D.ew[c] = ew[c]; D.eu[c] = eu[c]; D.ev[c] = ev[c]; }
     D.sdd = cb->sdd;
-    D.u0 = cb->off_u - 0.5 * (cb->nu - 1) * cb->du;
-    D.v0 = cb->off_v - 0.5 * (cb->nv - 1) * cb->dv;
+    D.off_u = cb->off_u;
+    D.off_v = cb->off_v;
     D.du = cb->du;
     D.dv = cb->dv;
     const double o[3] = {vol->ox, vol->oy, vol->oz}, sp[3] = {vol->sx, vol->sy, vol->sz};
-    for (int c = 0; c < 3; c++) { D.P[c] = (S[c] - o[c]) / sp[c] + 0.5; D.is[c] = 1.0 / sp[c]; }
+    for (int c = 0; c < 3; c++) {
+        D.S[c] = S[c];
+        D.o[c] = o[c];
+        D.s[c] = sp[c];
+        D.P[c] = (S[c] - o[c]) / sp[c] + 0.5;
+        D.is[c] = 1.0 / sp[c];
+    }
     D.n[0] = vol->nx; D.n[1] = vol->ny; D.n[2] = vol->nz;
     D.nu = cb->nu;
     D.nv = cb->nv;
