@@ -595,7 +595,7 @@ int eval_gradient_pipeline(const void* f0, const void* mean, const void* U, int 
     PCAS_LAUNCH(PCAS_K_WARP_PCA, s, first_warp(W, T, g, mean, U, dt, K, s));
     PCAS_LAUNCH(PCAS_K_DRR_SOLVER, s,
                 launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, 0, W.st, W.part_drr, W.part_adj,
-                                  T, 0ull, 0, occ_of(W, T), s));
+                                  T, 0ull, 0, occ_of(W, T), false, s));
     PCAS_LAUNCH(PCAS_K_RESID, s, launch_resid(W.pbuf, y, V, W.view, 1, W.rayt, W.st, W.part_res, s));
     PCAS_LAUNCH(PCAS_K_ADJ_GRAD, s,
                 launch_adjoint_grad(W.rayt, g, W.view, W.f0h, occ_of(W, T).f0m, mean, U, dt, K, step_setup, W.st,
@@ -619,7 +619,7 @@ int solve_host(const void* f0, const void* mean, const void* U, int dtype, int K
     PCAS_LAUNCH(PCAS_K_WARP_PCA, s, first_warp(W, T, g, mean, U, dtype, K, s));
     PCAS_LAUNCH(PCAS_K_DRR_SOLVER, s,
                 launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, 0, W.st, W.part_drr, W.part_adj,
-                                  T, 0ull, 0, occ_of(W, T), s));
+                                  T, 0ull, 0, occ_of(W, T), false, s));
     int iters = 0, flags[2] = {PH_RUNNING, -1};      // SolveState::phase, dense
     int& phase = flags[0];
     static_assert(offsetof(SolveState, dense) == offsetof(SolveState, phase) + sizeof(int), "read back together");
@@ -640,7 +640,7 @@ int solve_host(const void* f0, const void* mean, const void* U, int dtype, int K
                                                                 W.fpad4, W.fpad, occ_of(W, T), s));
             PCAS_LAUNCH(PCAS_K_DRR_BATCH, s,
                         launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, TRIAL_BATCH, W.st,
-                                          W.part_drr, W.part_adj, T, 0ull, 0, occ_of(W, T), s));
+                                          W.part_drr, W.part_adj, T, 0ull, 0, occ_of(W, T), false, s));
             PCAS_CUDA(cudaMemcpyAsync(flags, &W.st->phase, sizeof(flags), cudaMemcpyDeviceToHost, s));
             PCAS_CUDA(cudaStreamSynchronize(s));
             if (phase != PH_RUNNING) break;
@@ -886,7 +886,7 @@ int cost_grad_f0(const float* f0, const float* mean, const float* U, int K, cons
                                                         W.st->box[0], occ_of(W, T), s));
     PCAS_LAUNCH(PCAS_K_DRR_SOLVER, s,
                 launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, y, W.pbuf, 0, W.st, W.part_drr, W.part_adj,
-                                  T, 0ull, 0, occ_of(W, T), s));
+                                  T, 0ull, 0, occ_of(W, T), false, s));
     PCAS_LAUNCH(PCAS_K_RESID, s, launch_resid(W.pbuf, y, V, W.view, 1, W.rayt, W.st, W.part_res, s));
     if (dJdw)
         PCAS_LAUNCH(PCAS_K_ADJ_GRAD, s,
@@ -1624,7 +1624,7 @@ struct SideBranch {
     }
 };
 
-int capture_solve(pcas_solver s, cudaGraph_t graph, cudaStream_t cs, const float* y_src) {
+int capture_solve(pcas_solver s, cudaGraph_t graph, cudaStream_t cs, const float* y_src, bool crowd) {
     SideBranch side;
     if (side.init() != cudaSuccess) return fail(PCAS_ERR_CUDA, "graph build: stream/event creation failed");
     cudaStream_t cs2 = side.cs2;
@@ -1645,7 +1645,7 @@ int capture_solve(pcas_solver s, cudaGraph_t graph, cudaStream_t cs, const float
     PCAS_G(launch_fill_f0h(s->f0, s->dtype, g, W.f0h, s->tune.skip ? W.f0m : nullptr, &W.st->keep_f0h, cs));
     PCAS_G(first_warp(W, s->tune, g, s->mean, s->U, s->dtype, s->K, cs));
     PCAS_G(launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, s->y, W.pbuf, 0, W.st, W.part_drr, W.part_adj,
-                             s->tune, 0ull, 0, oc, cs));
+                             s->tune, 0ull, 0, oc, crowd, cs));
     k_ctrl_start<<<1, 1, 0, cs>>>(W.st, s->h_outer);
     PCAS_G(cudaGetLastError());
     cudaGraph_t outer_body;
@@ -1674,7 +1674,7 @@ int capture_solve(pcas_solver s, cudaGraph_t graph, cudaStream_t cs, const float
     PCAS_G(cudaStreamBeginCaptureToGraph(cs, inner_body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
     PCAS_G(launch_warp_batch(W.f0h, s->mean, s->U, s->dtype, s->K, W.st, g, W.view, W.fpad4, W.fpad, oc, cs));
     PCAS_G(launch_drr_solver(W.fpad, W.fpair, W.fpad4, g, V, W.view, s->y, W.pbuf, TRIAL_BATCH, W.st, W.part_drr,
-                             W.part_adj, s->tune, s->h_inner, 1, oc, cs));
+                             W.part_adj, s->tune, s->h_inner, 1, oc, crowd, cs));
     PCAS_G(cudaStreamEndCapture(cs, &done));
     return PCAS_OK;
 }
@@ -1856,7 +1856,7 @@ int pcas_solver_create(pcas_solver* out, const void* f0, const void* mean, const
         solver_free(s);
         return fail(PCAS_ERR_CUDA, "solver set-up failed: %s", cudaGetErrorString(e));
     }
-    rc = capture_solve(s, s->graph, cs, nullptr);
+    rc = capture_solve(s, s->graph, cs, nullptr, false);
     cudaStreamDestroy(cs);
     if (rc != PCAS_OK) { solver_free(s); return rc; }
     e = cudaGraphInstantiate(&s->exec, s->graph, 0);
@@ -2143,7 +2143,7 @@ int pcas_batch_create(pcas_batch* out, const pcas_solver* solvers, const float* 
         return fail(PCAS_ERR_CUDA, "batch set-up failed: %s", cudaGetErrorString(e));
     }
     int rc = PCAS_OK;
-    for (int i = 0; i < n && rc == PCAS_OK; i++) rc = capture_solve(solvers[i], b->graph, cs, y_src ? y_src[i] : nullptr);
+    for (int i = 0; i < n && rc == PCAS_OK; i++) rc = capture_solve(solvers[i], b->graph, cs, y_src ? y_src[i] : nullptr, n > 1);
     cudaStreamDestroy(cs);
     if (rc == PCAS_OK) {
         e = cudaGraphInstantiate(&b->exec, b->graph, 0);
