@@ -111,7 +111,7 @@ int drr_forward(const float* f, const pcas_vol* vol, const pcas_cb* cb, double s
  * Used to render measured images without the inverse crime of projecting
  * with the solver's own P; not on the solver path.  Ray geometry in double
  * precision, voxel traversal in 64-bit fixed point (2^-48 voxel), face crossings
- * to 2^-24 of a voxel layer, sums compensated (in double where float cannot hold
+ * to 2^-20 of a voxel layer or better, sums compensated (in double where float cannot hold
  * them), p rounded to float once.  A ray along a voxel face takes the voxel that
  * its position rounds down to.  f, p: device.  Asynchronous.
  * Errors: PCAS_ERR_INVALID_ARG for a NULL pointer, an invalid volume or
